@@ -64,8 +64,9 @@ typedef struct hf_params {
     double beta, dtau;   /* inverse temperature, Trotter step; L = round(beta / dtau)       */
     int n_matsubara;     /* Matsubara frequencies kept explicitly (paper: 500)              */
     int chains_per_site; /* independent Markov chains per inequivalent site                 */
-    int precision;       /* 0: FP64 sweeps; 1: FP32 sweeps + FP64 refresh; 2: FP32-pair     */
-                         /* ("double-float", 48-bit significand) sweeps + FP64 refresh      */
+    int precision;       /* 0: FP64 sweeps (updates in 64-bit fixed point up to dtau U = 3,  */
+                         /* in FP64 arithmetic above); 1: FP32 sweeps + FP64 refresh; 2:     */
+                         /* FP32-pair ("double-float", 48-bit significand) + FP64 refresh   */
     int refresh_every;   /* Dyson refresh after every refresh_every-th sweep of a chain     */
     int refresh_stagger; /* 0: a chain refreshes when its sweep counter n is a multiple of   */
                          /* refresh_every; 1: when n + site + chain is (site, chain = the    */
@@ -90,9 +91,10 @@ typedef struct hf_params {
     int delay_k;         /* delayed-update depth: 0/1 rank-1 Sherman-Morrison; 4, 8, 16, 32  */
                          /* (precision 2, one warp per chain): accepted flips gathered as    */
                          /* rank-k corrections                                              */
-    int team_warps;      /* FP32-pair sweeps: warps per Markov chain, 1, 2 or 4 (0: default  */
-                         /* 1 for L <= 32, 4 above); picked per L by the autotuner.  The     */
-                         /* FP64 sweeps accept the same values and choose their own width    */
+    int team_warps;      /* FP32-pair sweeps, and FP64 sweeps above dtau U = 3: warps per    */
+                         /* Markov chain, 1, 2 or 4 (0: default 1 for L <= 32, 4 above);     */
+                         /* picked per L by the autotuner.  The fixed-point FP64 sweeps      */
+                         /* accept the same values and choose their own width                */
     int bin_size;        /* measured sweeps per bin                                         */
     int max_bins;        /* bins kept per chain between clears                              */
     int n_warmup, n_measure;  /* sweeps per hf_rdmft_step                                  */

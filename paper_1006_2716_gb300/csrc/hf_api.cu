@@ -340,7 +340,8 @@ hf_status validate(const hf_params& p, std::string& err) {
     if (p.precision != 1) {
         const int tw = p.team_warps > 0 ? p.team_warps : hfk::qmc_default_team_warps(L);
         const size_t smem = (p.precision == 2) ? hfk::qmc_df64_smem_bytes(L, tw, p.delay_k)
-                                               : hfk::qmc_f64_smem_bytes(L);
+                            : hfk::qmc_f64_fixed(p.beta / L, p.U) ? hfk::qmc_f64_smem_bytes(L)
+                                                                  : hfk::qmc_f64_direct_smem_bytes(L, tw);
         if (smem > static_cast<size_t>(227) * 1024) {
             err = "team_warps / delay_k need " + std::to_string(smem) +
                   " bytes of shared memory per block (limit 232448); use more warps per chain or a "
@@ -502,6 +503,7 @@ hfk::QmcProblem make_problem(const hf_ctx& c, int n_warmup, int n_measure, int r
     q.max_bins = c.p.max_bins;
     q.refresh_first = refresh_first;
     q.team_warps = c.p.team_warps > 0 ? c.p.team_warps : hfk::qmc_default_team_warps(c.L);
+    q.fixed = c.p.precision == 0 ? hfk::qmc_f64_fixed(c.dtau, c.p.U) : 0;
     q.delay_k = c.p.delay_k > 1 ? c.p.delay_k : 1;
     q.gtau = c.gtau;
     q.G = c.G;
@@ -608,8 +610,8 @@ hf_status launch_sweeps(hf_ctx* c, int n_warmup, int n_measure, int refresh_firs
     b.nprob = 1;
     b.p[0] = make_problem(*c, n_warmup, n_measure, refresh_first);
     const int tw = b.p[0].team_warps;
-    const int cpb = c->p.precision == 2 ? hfk::qmc_df64_chains_per_block(tw) : hfk::qmc_f64_chains_per_block(c->L);
-    b.nblocks = (c->nchain + cpb - 1) / cpb;
+    const int cpb = hfk::qmc_df64_chains_per_block(tw);
+    b.nblocks = c->p.precision == 2 ? (c->nchain + cpb - 1) / cpb : hfk::qmc_f64_blocks(b.p[0]);
     cudaError_t e = (c->p.precision == 2)
                         ? hfk::launch_qmc_df64(b, hfk::qmc_df64_smem_bytes(c->L, tw, b.p[0].delay_k), c->stream)
                         : hfk::launch_qmc_f64(b, c->stream);
@@ -1294,8 +1296,8 @@ static hf_status enqueue_batch_qmc(hf_batch* b, int n_warmup, int n_measure, int
         qb.p[i].slot_mult = 1;   // several waves: the block scheduler balances them
         qb.p[i].block0 = blocks;
         const int tw = qb.p[i].team_warps;
-        const int cpb = c->p.precision == 2 ? hfk::qmc_df64_chains_per_block(tw) : hfk::qmc_f64_chains_per_block(c->L);
-        blocks += (c->nchain + cpb - 1) / cpb;
+        const int cpb = hfk::qmc_df64_chains_per_block(tw);
+        blocks += c->p.precision == 2 ? (c->nchain + cpb - 1) / cpb : hfk::qmc_f64_blocks(qb.p[i]);
         if (c->p.precision == 2) smem = std::max(smem, hfk::qmc_df64_smem_bytes(c->L, tw, qb.p[i].delay_k));
     }
     qb.nblocks = blocks;

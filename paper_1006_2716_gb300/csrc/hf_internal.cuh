@@ -72,7 +72,8 @@ struct QmcProblem {
     // single-precision path only: sweeps of this launch and the measured local range
     int nsweeps, meas_from, meas_to;
     int refresh_measure;  // refresh kernel: add a measurement after the refresh
-    int team_warps;       // FP32-pair sweeps: warps per chain (1, 2, 4; >= 2 for L > 32)
+    int team_warps;       // FP32-pair and direct FP64 sweeps: warps per chain (1, 2, 4; >= 2 for L > 32)
+    int fixed;            // FP64 sweeps: 1 fixed-point Green functions, 0 direct FP64 updates
     int site0;            // Philox site word = site0 + local site (served requests: the key's site)
     int delay_k;          // FP32-pair sweeps: delayed-update depth (<= 1: rank-1 updates)
     int refresh_stagger;  // 1: chain (site, c) refreshes when nsw + site + c = 0 mod refresh_every
@@ -111,8 +112,16 @@ __device__ __forceinline__ void drift_fold(unsigned int* drift, float v, bool co
     if (count) atomicAdd(drift + 1, 1u);
 }
 
-// FP64 sweeps: blocks of kBlock threads hold two chains (L <= 32) or one.
+// FP64 sweeps.  Up to dtau U = 3 (the strongest coupling of the configured workloads) with fixed-point
+// Green functions (k_qmc_f64.cu, blocks of kBlock threads hold two chains for L <= 32, else one),
+// above it with FP64 updates (k_qmc_f64_direct.cu, 4 / team_warps chains per block): one fixed-point
+// unit per row resolves the rows of G to FP64's accuracy and better at least up to there
+// (QmcProblem::fixed).
+constexpr double kFixedMaxDtauU = 3.0;
+inline int qmc_f64_fixed(double dtau, double U) { return dtau * U <= kFixedMaxDtauU * (1.0 + 1e-12) ? 1 : 0; }
 size_t qmc_f64_smem_bytes(int L);
+size_t qmc_f64_direct_smem_bytes(int L, int team_warps);
+int qmc_f64_direct_chains_per_block(int team_warps);
 // A second stream for part of a fused launch, and the events that tie it to the first.  Owned by
 // whoever launches (a batch, a server stream); not shared between threads.
 struct QmcFork {
@@ -122,9 +131,14 @@ struct QmcFork {
     void destroy();
 };
 bool qmc_f64_supported(int L);
-// Stream order on st; with f, problems of both shared-memory classes run side by side.
+// Stream order on st; with f, fixed-point problems of both shared-memory classes run side by side.
 cudaError_t launch_qmc_f64(const QmcBatch& b, cudaStream_t st, const QmcFork* f = nullptr);
+cudaError_t launch_qmc_f64_direct(const QmcBatch& b, cudaStream_t st);
 int qmc_f64_chains_per_block(int L);
+inline int qmc_f64_blocks(const QmcProblem& p) {
+    const int cpb = p.fixed ? qmc_f64_chains_per_block(p.L) : qmc_f64_direct_chains_per_block(p.team_warps);
+    return (p.nchain + cpb - 1) / cpb;
+}
 int qmc_default_team_warps(int L);
 
 // FP32-pair ("double-float") sweeps with FP64 refresh: the FP64 kernel's L set, blocks of kBlock

@@ -286,6 +286,7 @@ hf_status start_launch(hf_srv* S, Launch& Lh) {
         q.max_bins = S->nb;
         q.refresh_first = 1;
         q.team_warps = p.team_warps > 0 ? p.team_warps : hfk::qmc_default_team_warps(L);
+        q.fixed = p.precision == 0 ? hfk::qmc_f64_fixed(dtau, j.req.U) : 0;
         q.delay_k = 1;
         if (L > 32 && q.team_warps == 1) q.team_warps = 2;
         q.gtau = b.gtau;
@@ -297,8 +298,8 @@ hf_status start_launch(hf_srv* S, Launch& Lh) {
         q.acc = b.acc;
         q.bins = b.bins;
         q.status = b.status;
-        const int cpb = p.precision == 2 ? hfk::qmc_df64_chains_per_block(q.team_warps) : hfk::qmc_f64_chains_per_block(L);
-        blocks += (cps + cpb - 1) / cpb;
+        const int cpb = hfk::qmc_df64_chains_per_block(q.team_warps);
+        blocks += p.precision == 2 ? (cps + cpb - 1) / cpb : hfk::qmc_f64_blocks(q);
         if (p.precision == 2) smem = std::max(smem, hfk::qmc_df64_smem_bytes(L, q.team_warps, 1));
     }
     qb.nblocks = blocks;

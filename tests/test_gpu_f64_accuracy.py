@@ -1,0 +1,84 @@
+"""Accuracy of the FP64 sweeps between two refreshes: after some sweeps of Sherman-Morrison
+updates, G is compared with the same updates in 113-bit arithmetic (green_error.cpp), beside what
+rank-1 updates in FP64 reach from the same matrices."""
+import ctypes as C
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+import oracle as o
+from paper_1006_2716_gb300 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def hf():
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    from paper_1006_2716_gb300 import build as B
+
+    B.build()
+    from paper_1006_2716_gb300 import hf as H
+
+    return H
+
+
+@pytest.fixture(scope="module")
+def helper(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("green") / "libgreen_error.so")
+    subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-fPIC", "-shared", "-pthread",
+                    "-o", so, os.path.join(HERE, "green_error.cpp")], check=True)
+    return C.CDLL(so)
+
+
+def sweep_errors(hf, helper, L, U, dtau, chains, nsweep):
+    """[chains][2] errors of the library's G and of FP64 rank-1 updates after nsweep sweeps from a
+    refreshed state (relative to max|G|), over one random bath per 8 chains."""
+    beta, cps = L * dtau, 8
+    err = np.zeros((chains, 2))
+    err64 = np.zeros((chains, 2))
+    _, lam = o.constants(beta, U, L)
+    for c0 in range(0, chains, cps):
+        cfg = dict(wl.CONFIGS["square6"], Lx=1, Ly=1, beta=beta, dtau=dtau, U=U, chains_per_site=cps,
+                   refresh_every=1000, bin_size=4, max_bins=1, seed=99 + c0, n_matsubara=4)
+        ctx = hf.Context(hf.make_params(cfg))
+        bath = wl.random_baths(31 * L + c0, 1, beta, L)[0]
+        for sp in range(2):
+            hf.hf_set_g0(ctx.handle, 0, sp, bath[sp])
+        hf.hf_sweep(ctx.handle, 10, 0, 1)
+        hf.hf_sweep(ctx.handle, 0, 0, 1)
+        s0, _ = hf.hf_get_fields(ctx.handle, cps, L)
+        G0 = np.array([hf.hf_get_green(ctx.handle, c, L) for c in range(cps)])
+        hf.hf_sweep(ctx.handle, nsweep, 0, 0)
+        s1, _ = hf.hf_get_fields(ctx.handle, cps, L)
+        G1 = np.array([hf.hf_get_green(ctx.handle, c, L) for c in range(cps)])
+        ctx.close()
+        u = np.array([[[o.uniform(cfg["seed"], 0, c, 10 + w, l) for l in range(L)]
+                       for w in range(nsweep)] for c in range(cps)])
+        e, e64, s = np.zeros((cps, 2)), np.zeros((cps, 2)), np.zeros((cps, L), dtype=np.int8)
+        dp = lambda a: a.ctypes.data_as(C.POINTER(C.c_double))
+        i8 = lambda a: a.ctypes.data_as(C.POINTER(C.c_int8))
+        s0 = np.ascontiguousarray(s0, dtype=np.int8)
+        helper.green_errors(L, cps, nsweep, C.c_double(np.exp(-2 * lam) - 1), C.c_double(np.exp(2 * lam) - 1),
+                            dp(G0), i8(s0), dp(u), dp(G1), dp(e), dp(e64), i8(s))
+        assert np.array_equal(s, s1)
+        err[c0:c0 + cps], err64[c0:c0 + cps] = e, e64
+    return err, err64
+
+
+@pytest.mark.parametrize("L,U", [(8, 120.0), (16, 80.0), (20, 12.1), (24, 32.0), (64, 40.0)])
+def test_strong_coupling_updates_are_fp64s(hf, helper, L, U):
+    """dtau U > 3: G is as close to exact updates as FP64 rank-1 updates are.  The two sides round
+    in a different order, and one interval's error scatters around the other's by the spread of
+    single roundings, so the worst and the 90 % mark over 128 matrices agree within a factor of
+    eight; 1e-15 for intervals without a flip."""
+    err, err64 = sweep_errors(hf, helper, L, U, 0.25, 64, 10)
+    for q in (0.9, 1.0):
+        assert np.quantile(err, q) <= 8 * np.quantile(err64, q) + 1e-15, (q, np.quantile(err, q), np.quantile(err64, q))
