@@ -1,15 +1,19 @@
 """Autotuner of the sweep kernels: for each slice count L, the arithmetic form of the FP64-class
-sweeps (0 = FP64, 2 = FP32 pairs with FP64 refresh; both meet the FP64 parity bar), the number of
-warps per Markov chain and the delayed-update depth k in {1, 4, 8, 16, 32} (FP32-pair form) that
-give the most proposals per second on this GPU.
+sweeps (0 = FP64, 2 = FP32 pairs, a 48-bit significand, with FP64 refresh), the number of warps per
+Markov chain (FP32-pair form, and FP64 form above dtau U = 3: up to there the fixed-point kernel
+chooses its own) and the delayed-update depth k in {1, 4, 8, 16, 32} (FP32-pair form) that give the
+most proposals per second on this GPU.
 
 Each candidate runs the real fused sweep kernel and is timed with CUDA events on the context
 stream (hf_get_timings): ``tune_workload`` runs whole RDMFT iterations of a workload configuration
 (its own baths, measurement cadence and acceptance rates); ``tune`` probes a synthetic
-single-impurity problem per L.  Results are cached per GPU name in ``_build/autotune.json``.
+single-impurity problem per L.  Results are cached per GPU name and kernel sources in
+``_build/autotune.json``.
 """
 from __future__ import annotations
 
+import functools
+import hashlib
 import json
 import os
 
@@ -18,10 +22,22 @@ import numpy as np
 from . import hf
 from . import workloads as wl
 
-_CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_build", "autotune.json")
-
+_HERE = os.path.dirname(os.path.abspath(__file__))
+_CACHE = os.path.join(_HERE, "_build", "autotune.json")
+_SOURCES = ("k_qmc_f64.cu", "k_qmc_f64_direct.cu", "k_qmc_df64.cu", "qmc_common.cuh", "hf_internal.cuh")
 
 DELAYS = (1, 4, 8, 16, 32)
+FIXED_MAX_DTAU_U = 3.0      # the fixed-point FP64 kernel's couplings (kFixedMaxDtauU of the library)
+
+
+@functools.lru_cache(maxsize=None)
+def sources_digest():
+    """Digest of the sweep kernels' sources: a timing is kept for the kernels it was taken of."""
+    h = hashlib.sha256()
+    for f in _SOURCES:
+        with open(os.path.join(_HERE, "csrc", f), "rb") as fh:
+            h.update(fh.read())
+    return h.hexdigest()[:12]
 
 
 def _fits(L, tw, k):
@@ -32,22 +48,30 @@ def _fits(L, tw, k):
     return (4 // tw) * (team + delayed) <= 227 * 1024
 
 
-def candidates(L, forms=(0, 2)):
+def candidates(L, forms=(0, 2), dtau_U=None):
     """(form, warps per chain, delay depth) triples.  Delayed updates exist in the FP32-pair form
-    and run with one warp per chain (L <= 32)."""
+    and run with one warp per chain (L <= 32).  Without dtau_U every triple the library accepts; with
+    it those that differ: the fixed-point FP64 kernel runs the same launch for every width, so it is
+    offered once, with the library's default width."""
     tws = (1, 2, 4) if L <= 32 else (2, 4)
+    fixed = dtau_U is not None and dtau_U <= FIXED_MAX_DTAU_U * (1.0 + 1e-12)
     out = []
     for f in forms:
         for tw in tws:
+            if f == 0 and fixed and tw != (1 if L <= 32 else 4):
+                continue
             for k in (DELAYS if (f == 2 and tw == 1) else (1,)):
                 if f == 0 or _fits(L, tw, k):
                     out.append((f, tw, k))
     return out
 
 
+_PROBE_U, _PROBE_DTAU = 8.0, 0.25
+
+
 def _probe(L, chains, form, tw, k, sweeps, device, stream):
-    beta = 0.25 * L
-    cfg = dict(Lx=1, Ly=1, geometry=0, U=8.0, V0=0.0, mu=4.0, beta=beta, dtau=0.25,
+    beta = _PROBE_DTAU * L
+    cfg = dict(Lx=1, Ly=1, geometry=0, U=_PROBE_U, V0=0.0, mu=4.0, beta=beta, dtau=_PROBE_DTAU,
                n_matsubara=4, chains_per_site=chains, precision=form, team_warps=tw, delay_k=k,
                refresh_every=10, bin_size=max(1, sweeps), max_bins=1, n_warmup=0,
                n_measure=sweeps, seed=12345)
@@ -94,10 +118,10 @@ def tune_workload(name, cfg, forms=(0, 2), iterations=2, device="cuda:0", stream
             cache = json.load(open(_CACHE))
         except (OSError, ValueError):
             cache = {}
-    key = "%s|%s|L=%d|forms=%s|v4" % (gpu, name, L, ",".join(map(str, forms)))
+    key = "%s|%s|L=%d|forms=%s|%s" % (gpu, name, L, ",".join(map(str, forms)), sources_digest())
     if key not in cache:
         table = {}
-        for form, tw, k in candidates(L, forms):
+        for form, tw, k in candidates(L, forms, cfg["dtau"] * cfg["U"]):
             table["%d/%d/%d" % (form, tw, k)] = _probe_workload(cfg, form, tw, k, iterations,
                                                                 device, stream)
         pick = min(table, key=table.get)
@@ -123,10 +147,10 @@ def tune(Ls, chains, forms=(0, 2), sweeps=30, device="cuda:0", stream=None, use_
             cache = {}
     out = {}
     for L in Ls:
-        key = "%s|L=%d|chains=%d|forms=%s|v3" % (name, L, chains, ",".join(map(str, forms)))
+        key = "%s|L=%d|chains=%d|forms=%s|%s" % (name, L, chains, ",".join(map(str, forms)), sources_digest())
         if key not in cache:
             table = {}
-            for form, tw, k in candidates(L, forms):
+            for form, tw, k in candidates(L, forms, _PROBE_DTAU * _PROBE_U):
                 table["%d/%d/%d" % (form, tw, k)] = _probe(L, chains, form, tw, k, sweeps, device,
                                                            stream)
             pick = min(table, key=table.get)
