@@ -104,7 +104,11 @@ typedef struct hf_params {
     void* cuda_stream;   /* cudaStream_t used for every device operation                    */
 } hf_params;
 
-/* Bytes of device workspace hf_init needs for *p (*bytes set on HF_OK). */
+/* Bytes of device workspace of *p (*bytes set on HF_OK).  They hold band buffers for the fewest
+ * launches per lattice step: up to 24 GiB in the blocked band form, up to 8 GiB in the window form
+ * where an SM holds several windows (band half-widths up to 115), else 1 GiB.  hf_init of a
+ * window-form lattice also takes less, down to 1 GiB of band buffers (or all it needs, if that is
+ * less), and then uses what it is given; the results are the same. */
 hf_status hf_workspace_size(const hf_params* p, size_t* bytes);
 
 /* Host only, no device work: the lattice *p describes (after the same validation as hf_init).
@@ -119,12 +123,13 @@ hf_status hf_lattice_info(const hf_params* p, int* N, int* n_sites, int* band, i
 
 /* Validate *p, build the lattice (eq. 1) and its point-group orbits (C4v in two dimensions,
  * the cubic group for the box, the planar group with the layer translations for the slab), lay
- * the state out in the caller's device workspace d_ws (ws_bytes >= hf_workspace_size), draw the
+ * the state out in the caller's device workspace d_ws (ws_bytes >= hf_workspace_size, or the smaller
+ * sizes described there), draw the
  * initial Ising fields of every chain and seed Sigma_{i,sigma}(i w_n) = U/2 - sigma h_seed
  * eps_i.  *out receives a host handle released by hf_free.  HF_EINVAL for invalid parameters,
  * including a lattice whose band half-width in the lattice step's band order (periodic axes
  * folded) exceeds 840, the widest band the blocked band form keeps buffers for; HF_ENOMEM for
- * a workspace smaller than hf_workspace_size. */
+ * a workspace smaller than the smallest accepted. */
 hf_status hf_init(const hf_params* p, void* d_ws, size_t ws_bytes, hf_ctx** out);
 
 /* Number of inequivalent sites, chains, L, lattice sites N (any pointer may be NULL). */

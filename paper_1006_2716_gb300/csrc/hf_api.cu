@@ -425,12 +425,29 @@ size_t layout(hf_ctx& c, void* base) {
 // radius-40 disc, where an SM holds several windows, else 1), split evenly over the launches: each
 // launch ends with a partial wave (1 GiB, 162 matrices, took that disc seven launches of one wave
 // of single blocks and a nearly empty second one each: 558 ms against 276).
-void set_lattice_batch(hf_ctx& c, int gib) {
+size_t lattice_cap(const hf_ctx& c, int gib) {
     const size_t per = hfk::lattice_scratch_per_matrix(c.lat.N, c.lat.b);
+    return std::max<size_t>(1, (static_cast<size_t>(gib) << 30) / (per ? per : 1));
+}
+void set_lattice_batch(hf_ctx& c, size_t cap) {
     const size_t nq = static_cast<size_t>(c.lat.gdn.empty() ? 2 : 1) * c.nw;
-    const size_t cap = std::max<size_t>(1, (static_cast<size_t>(gib) << 30) / (per ? per : 1));
     const size_t nl = (nq + cap - 1) / cap;
     c.lat_batch = static_cast<int>((nq + nl - 1) / nl);
+}
+
+// A workspace of ws_bytes, smaller than the full one: the fewest lattice launches whose band buffers
+// fit it (window form; at least those of 1 GiB, the smallest accepted).  Returns the bytes needed.
+size_t fit_lattice_batch(hf_ctx& c, size_t ws_bytes) {
+    size_t hi = lattice_cap(c, 8);       // layouts of lo fit (or are the smallest), larger caps are tried
+    size_t lo = std::min(lattice_cap(c, 1), hi);
+    while (lo < hi) {
+        const size_t mid = lo + (hi - lo + 1) / 2;
+        set_lattice_batch(c, mid);
+        if (layout(c, nullptr) <= ws_bytes) lo = mid;
+        else hi = mid - 1;
+    }
+    set_lattice_batch(c, lo);
+    return layout(c, nullptr);
 }
 
 hf_status setup_sizes(hf_ctx& c, const hf_params* p) {
@@ -457,7 +474,7 @@ hf_status setup_sizes(hf_ctx& c, const hf_params* p) {
     c.nsite = static_cast<int>(c.lat.rep.size());
     c.nchain = c.nsite * p->chains_per_site;
     c.nw = p->n_matsubara;
-    set_lattice_batch(c, c.lat_wide ? 24 : hfk::lattice_windows_share_sm(c.lat.b) ? 8 : 1);
+    set_lattice_batch(c, lattice_cap(c, c.lat_wide ? 24 : hfk::lattice_windows_share_sm(c.lat.b) ? 8 : 1));
     return HF_OK;
 }
 
@@ -720,10 +737,7 @@ hf_status hf_init(const hf_params* p, void* d_ws, size_t ws_bytes, hf_ctx** out)
     hf_status st = setup_sizes(*c, p);
     if (st != HF_OK) { delete c; return st; }
     size_t need = layout(*c, nullptr);
-    if (d_ws && ws_bytes < need && !c->lat_wide) {   // a smaller workspace takes more lattice launches
-        set_lattice_batch(*c, 1);
-        need = layout(*c, nullptr);
-    }
+    if (d_ws && ws_bytes < need && !c->lat_wide) need = fit_lattice_batch(*c, ws_bytes);
     if (!d_ws || ws_bytes < need) {
         delete c;
         return fail(nullptr, HF_ENOMEM, "workspace of " + std::to_string(ws_bytes) +
