@@ -340,7 +340,7 @@ hf_status validate(const hf_params& p, std::string& err) {
     if (p.precision != 1) {
         const int tw = p.team_warps > 0 ? p.team_warps : hfk::qmc_default_team_warps(L);
         const size_t smem = (p.precision == 2) ? hfk::qmc_df64_smem_bytes(L, tw, p.delay_k)
-                            : hfk::qmc_f64_fixed(p.beta / L, p.U) ? hfk::qmc_f64_smem_bytes(L)
+                            : hfk::qmc_f64_row_bits(L, p.beta / L, p.U) ? hfk::qmc_f64_smem_bytes(L)
                                                                   : hfk::qmc_f64_direct_smem_bytes(L, tw);
         if (smem > static_cast<size_t>(227) * 1024) {
             err = "team_warps / delay_k need " + std::to_string(smem) +
@@ -520,7 +520,7 @@ hfk::QmcProblem make_problem(const hf_ctx& c, int n_warmup, int n_measure, int r
     q.max_bins = c.p.max_bins;
     q.refresh_first = refresh_first;
     q.team_warps = c.p.team_warps > 0 ? c.p.team_warps : hfk::qmc_default_team_warps(c.L);
-    q.fixed = c.p.precision == 0 ? hfk::qmc_f64_fixed(c.dtau, c.p.U) : 0;
+    q.row_bits = c.p.precision == 0 ? hfk::qmc_f64_row_bits(c.L, c.dtau, c.p.U) : 0;
     q.delay_k = c.p.delay_k > 1 ? c.p.delay_k : 1;
     q.gtau = c.gtau;
     q.G = c.G;

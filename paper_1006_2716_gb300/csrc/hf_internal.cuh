@@ -73,7 +73,7 @@ struct QmcProblem {
     int nsweeps, meas_from, meas_to;
     int refresh_measure;  // refresh kernel: add a measurement after the refresh
     int team_warps;       // FP32-pair and direct FP64 sweeps: warps per chain (1, 2, 4; >= 2 for L > 32)
-    int fixed;            // FP64 sweeps: 1 fixed-point Green functions, 0 direct FP64 updates
+    int row_bits;         // FP64 sweeps: bits of a fixed-point row, 0: updates in FP64 arithmetic
     int site0;            // Philox site word = site0 + local site (served requests: the key's site)
     int delay_k;          // FP32-pair sweeps: delayed-update depth (<= 1: rank-1 updates)
     int refresh_stagger;  // 1: chain (site, c) refreshes when nsw + site + c = 0 mod refresh_every
@@ -114,11 +114,26 @@ __device__ __forceinline__ void drift_fold(unsigned int* drift, float v, bool co
 
 // FP64 sweeps.  Up to dtau U = 3 (the strongest coupling of the configured workloads) with fixed-point
 // Green functions (k_qmc_f64.cu, blocks of kBlock threads hold two chains for L <= 32, else one),
-// above it with FP64 updates (k_qmc_f64_direct.cu, 4 / team_warps chains per block): one fixed-point
-// unit per row resolves the rows of G to FP64's accuracy and better at least up to there
-// (QmcProblem::fixed).
-constexpr double kFixedMaxDtauU = 3.0;
-inline int qmc_f64_fixed(double dtau, double U) { return dtau * U <= kFixedMaxDtauU * (1.0 + 1e-12) ? 1 : 0; }
+// above it with FP64 updates (k_qmc_f64_direct.cu, 4 / team_warps chains per block).
+//
+// Bits of a fixed-point row (QmcProblem::row_bits; 0: FP64 updates).  One unit per row resolves its
+// largest elements better than FP64 and its smallest ones worse, and the ratio between them grows
+// with e^{dtau U} and with L.  Error of G (relative to its maximum) after ten sweeps, fixed point over
+// FP64 rank-1 updates, at the marks that 90 % and 99 % of 1536 or 3072 intervals stay below (a CPU
+// restatement of both beside 113-bit updates, random baths, dtau = 0.25):
+//     L, U      57 bits        58 bits        59 bits
+//     16, 4     0.38, 0.52     0.21, 0.36     0.12, 0.13
+//     32, 4     0.66, 1.1      0.37, 0.60     0.18, 0.24
+//     32, 8     1.0,  1.5      0.55, 0.92     0.27, 0.34
+//     32, 12    1.4,  2.8      0.71, 1.4      0.37, 0.79
+//     64, 12    2.7,  5.4      1.4,  2.9      0.63, 1.0
+// 57 bits up to L = 32 and dtau U = 1, 59 beyond.  At L = 32, U = 8 the latter give one flip in ten new
+// units, 57 bits one in a hundred.
+constexpr double kFixedMaxDtauU = 3.0, kFewBitsMaxDtauU = 1.0;
+inline int qmc_f64_row_bits(int L, double dtau, double U) {
+    if (dtau * U > kFixedMaxDtauU * (1.0 + 1e-12)) return 0;
+    return L <= 32 && dtau * U <= kFewBitsMaxDtauU * (1.0 + 1e-12) ? 57 : 59;
+}
 size_t qmc_f64_smem_bytes(int L);
 size_t qmc_f64_direct_smem_bytes(int L, int team_warps);
 int qmc_f64_direct_chains_per_block(int team_warps);
@@ -136,7 +151,7 @@ cudaError_t launch_qmc_f64(const QmcBatch& b, cudaStream_t st, const QmcFork* f 
 cudaError_t launch_qmc_f64_direct(const QmcBatch& b, cudaStream_t st);
 int qmc_f64_chains_per_block(int L);
 inline int qmc_f64_blocks(const QmcProblem& p) {
-    const int cpb = p.fixed ? qmc_f64_chains_per_block(p.L) : qmc_f64_direct_chains_per_block(p.team_warps);
+    const int cpb = p.row_bits ? qmc_f64_chains_per_block(p.L) : qmc_f64_direct_chains_per_block(p.team_warps);
     return (p.nchain + cpb - 1) / cpb;
 }
 int qmc_default_team_warps(int L);

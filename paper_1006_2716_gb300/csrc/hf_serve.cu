@@ -286,7 +286,7 @@ hf_status start_launch(hf_srv* S, Launch& Lh) {
         q.max_bins = S->nb;
         q.refresh_first = 1;
         q.team_warps = p.team_warps > 0 ? p.team_warps : hfk::qmc_default_team_warps(L);
-        q.fixed = p.precision == 0 ? hfk::qmc_f64_fixed(dtau, j.req.U) : 0;
+        q.row_bits = p.precision == 0 ? hfk::qmc_f64_row_bits(L, dtau, j.req.U) : 0;
         q.delay_k = 1;
         if (L > 32 && q.team_warps == 1) q.team_warps = 2;
         q.gtau = b.gtau;
