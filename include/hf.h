@@ -41,7 +41,8 @@ typedef enum {
     HF_ENOMEM = -2,    /* workspace too small                                          */
     HF_ECUDA = -3,     /* a CUDA runtime call failed                                   */
     HF_ETIMEOUT = -4,  /* a bounded device wait ran out                                */
-    HF_ENUMERIC = -5,  /* singular Dyson matrix or non-finite value detected on device */
+    HF_ENUMERIC = -5,  /* singular Dyson matrix or non-finite value detected on device; the */
+                       /* chain's G and observables are NaN until a refresh gives a finite G */
     HF_EBUSY = -6,     /* no free slot / resource                                      */
     HF_ENOTREADY = -7  /* requested result is not available yet                        */
 } hf_status;

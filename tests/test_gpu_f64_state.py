@@ -1,0 +1,69 @@
+"""The FP64 sweeps' state between launches: non-finite matrices."""
+import numpy as np
+import pytest
+
+from paper_1006_2716_gb300 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+LS = [8, 12, 16, 20, 24, 32, 40, 48, 64]
+
+
+@pytest.fixture(scope="module")
+def hf():
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    from paper_1006_2716_gb300 import build as B
+
+    B.build()
+    from paper_1006_2716_gb300 import hf as H
+
+    return H
+
+
+def _context(hf, L, U, n=6, cps=4, bin_size=2):
+    cfg = dict(wl.CONFIGS["square6"], Lx=n, Ly=n, beta=0.25 * L, dtau=0.25, U=U, chains_per_site=cps,
+               refresh_every=10, bin_size=bin_size, max_bins=4, n_matsubara=4, seed=17)
+    ctx = hf.Context(hf.make_params(cfg))
+    baths = wl.random_baths(3 * L, ctx.n_sites, 0.25 * L, L)
+    for i in range(ctx.n_sites):
+        for sp in range(2):
+            hf.hf_set_g0(ctx.handle, i, sp, baths[i, sp])
+    return ctx
+
+
+def _state(hf, ctx):
+    hf.hf_sync(ctx.handle)
+    G = np.array([hf.hf_get_green(ctx.handle, c, ctx.L) for c in range(ctx.n_chains)])
+    obs = [hf.hf_measure(ctx.handle, i, ctx.L) for i in range(ctx.n_sites)]
+    fields, count = hf.hf_get_fields(ctx.handle, ctx.n_chains, ctx.L)
+    acc = hf.hf_get_accepts(ctx.handle, ctx.n_chains)
+    return [G, fields, count, acc] + [np.concatenate([np.ravel(x) for x in ob]) for ob in obs]
+
+
+@pytest.mark.parametrize("L", [8, 32, 40, 64])
+def test_a_matrix_that_is_not_finite_stays_so(hf, L):
+    """A zero bath has no inverse: the launch reports it, a further launch without a refresh reports it
+    again, and the matrix and the observables of that spin show it until a refresh finds a good
+    bath."""
+    ctx = _context(hf, L, 8.0, n=1, cps=2)
+    good = hf.hf_get_g0(ctx.handle, 1, L)[0]
+    hf.hf_set_g0(ctx.handle, 0, 1, np.zeros(L))
+    for k in range(3):
+        hf.hf_sweep(ctx.handle, 0, 4 if k else 0, 1 if k == 0 else 0)
+        with pytest.raises(hf.HFError) as e:
+            hf.hf_sync(ctx.handle)
+        assert e.value.status == hf.HF_ENUMERIC
+        G = hf.hf_get_green(ctx.handle, 0, L)
+        assert np.all(np.isfinite(G[0])) and not np.any(np.isfinite(G[1]))
+    gtau, n, d, m, _ = hf.hf_measure(ctx.handle, 0, L)
+    assert np.all(np.isfinite(gtau[:L])) and np.all(np.isnan(gtau[L:]))
+    assert np.isfinite(n[0]) and np.isnan(n[1]) and np.isnan(d) and np.isnan(m)
+    assert not hf.hf_get_accepts(ctx.handle, 2).any()
+    hf.hf_set_g0(ctx.handle, 0, 1, good[1])
+    hf.hf_clear_measurements(ctx.handle)
+    hf.hf_sweep(ctx.handle, 0, 4, 1)
+    assert all(np.all(np.isfinite(x)) for x in _state(hf, ctx))
+    ctx.close()
