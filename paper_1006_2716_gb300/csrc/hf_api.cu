@@ -249,6 +249,8 @@ struct hf_ctx {
     std::string err;
     // device state
     double* gtau = nullptr;         // [nsite][2][L]
+    int16_t* G_lo = nullptr;        // [nchain][2][L*L] fixed-point sweeps: the part of G that FP64 leaves out
+    int* G_unit = nullptr;          // [nchain][2][L] and its rows' units
     double* G = nullptr;            // [nchain][2][L*L]
     float* Gf = nullptr;            // [nchain][2][L*L] (precision 1)
     double* g0inv = nullptr;        // [nsite][2][L*L] inverse bath matrices
@@ -380,6 +382,9 @@ size_t layout(hf_ctx& c, void* base) {
     const int L = c.L, ns = c.nsite, nc = c.nchain, nw = c.nw, N = c.lat.N, bw = c.lat.b + 1;
     c.gtau = cv.take<double>(static_cast<size_t>(ns) * 2 * L);
     c.G = cv.take<double>(static_cast<size_t>(nc) * 2 * L * L);
+    const bool fixed = c.p.precision == 0 && hfk::qmc_f64_row_bits(L, c.p.beta / L, c.p.U) > 0;
+    c.G_lo = fixed ? cv.take<int16_t>(static_cast<size_t>(nc) * 2 * L * L) : nullptr;
+    c.G_unit = fixed ? cv.take<int>(static_cast<size_t>(nc) * 2 * L) : nullptr;
     c.Gf = c.p.precision == 1 ? cv.take<float>(static_cast<size_t>(nc) * 2 * L * L) : nullptr;
     c.g0inv = cv.take<double>(static_cast<size_t>(ns) * 2 * L * L);
     c.s = cv.take<int8_t>(static_cast<size_t>(nc) * L);
@@ -524,6 +529,8 @@ hfk::QmcProblem make_problem(const hf_ctx& c, int n_warmup, int n_measure, int r
     q.delay_k = c.p.delay_k > 1 ? c.p.delay_k : 1;
     q.gtau = c.gtau;
     q.G = c.G;
+    q.G_lo = c.G_lo;
+    q.G_unit = c.G_unit;
     q.Gf = c.Gf;
     q.g0inv = c.g0inv;
     q.s = c.s;

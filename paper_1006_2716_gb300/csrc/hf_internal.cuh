@@ -84,6 +84,8 @@ struct QmcProblem {
     const double* gtau;   // [nsite][2][L]  bath g~0(tau_m)
     double* g0inv;        // [nsite][2][L*L] inverse bath matrices (rebuilt with the bath)
     double* G;            // [nchain][2][L*L] (FP64 state, or FP64 scratch of the FP32 path)
+    int16_t* G_lo;        // [nchain][2][L*L], G_unit [nchain][2][L]: what G leaves out of the fixed-point
+    int* G_unit;          // state and its rows' units, for the next launch; or nullptr (no next launch)
     float* Gf;            // [nchain][2][L*L] FP32 state (precision 1) or nullptr
     int8_t* s;            // [nchain][L]
     uint32_t* nsw;        // [nchain] sweeps done

@@ -1,4 +1,4 @@
-"""The FP64 sweeps' state between launches: non-finite matrices."""
+"""The FP64 sweeps' state between launches: runs split off a refresh, non-finite matrices."""
 import numpy as np
 import pytest
 
@@ -41,6 +41,20 @@ def _state(hf, ctx):
     fields, count = hf.hf_get_fields(ctx.handle, ctx.n_chains, ctx.L)
     acc = hf.hf_get_accepts(ctx.handle, ctx.n_chains)
     return [G, fields, count, acc] + [np.concatenate([np.ravel(x) for x in ob]) for ob in obs]
+
+
+@pytest.mark.parametrize("L", LS)
+def test_a_run_in_several_launches_is_the_run_in_one(hf, L, U):
+    """Split off the refreshes (after sweeps 10, 20 of a chain) and within a bin: bit for bit."""
+    out = []
+    for launches in (((15, 8),), ((7, 0), (8, 3), (0, 5)), ((13, 0), (1, 0), (1, 1), (0, 7))):
+        ctx = _context(hf, L, U)
+        for k, (w, m) in enumerate(launches):
+            hf.hf_sweep(ctx.handle, w, m, 1 if k == 0 else 0)
+        out.append(_state(hf, ctx))
+        ctx.close()
+    for other in out[1:]:
+        assert all(np.array_equal(a, b) for a, b in zip(out[0], other))
 
 
 @pytest.mark.parametrize("L", [8, 32, 40, 64])
