@@ -1,4 +1,7 @@
-"""The FP64 sweeps' state between launches: runs split off a refresh, non-finite matrices."""
+"""The FP64 sweeps' state between launches: runs split off a refresh, non-finite matrices, and what one
+measurement adds."""
+import math
+
 import numpy as np
 import pytest
 
@@ -80,4 +83,21 @@ def test_a_matrix_that_is_not_finite_stays_so(hf, L):
     hf.hf_clear_measurements(ctx.handle)
     hf.hf_sweep(ctx.handle, 0, 4, 1)
     assert all(np.all(np.isfinite(x)) for x in _state(hf, ctx))
+    ctx.close()
+
+
+@pytest.mark.parametrize("L,U", [(16, 12.0), (32, 12.0), (40, 8.0), (64, 12.0)])
+def test_a_measurement_is_the_sum_over_g(hf, L, U):
+    """One measurement against the exact sums over the stored G: every element of that is rounded to
+    2^-53 of itself, and so are the result and the sums behind n."""
+    ctx = _context(hf, L, U, n=14, cps=1, bin_size=1)
+    hf.hf_sweep(ctx.handle, 7, 1, 1)
+    for i in range(ctx.n_sites):
+        got = hf.hf_measure(ctx.handle, i, L)[0]
+        G = hf.hf_get_green(ctx.handle, i, L)
+        for sp in range(2):
+            for m in range(L):
+                x = [(1.0 if l + m < L else -1.0) * G[sp, (l + m) % L, l] for l in range(L)]
+                tol = 4 * 2.0 ** -53 * math.fsum(map(abs, x)) / L
+                assert abs(got[sp * L + m] - math.fsum(x) / L) <= tol, (i, sp, m)
     ctx.close()
