@@ -153,7 +153,8 @@ hf_status hf_set_g0(hf_ctx* ctx, int site, int spin, const double* g0_tau);
  * from the current bath and fields (in FP64, as G = [g0^{-1} e^V - (e^V - 1)]^{-1}).  Per chain: sweep number w uses Philox counter
  * (w, l, chain, site); after the sweep the chain's counter advances and a Dyson refresh runs
  * when it is a multiple of refresh_every; measured sweeps then add to the current bin.  A run split
- * over several calls (refresh_first = 0 after the first) is the run in one call bit for bit. */
+ * over several calls (refresh_first = 0 after the first) is the run in one call bit for bit
+ * (precision 0). */
 hf_status hf_sweep(hf_ctx* ctx, int n_warmup, int n_measure, int refresh_first);
 
 /* Zero all measurement bins and counters (the next measured sweep starts bin 0), the drift
