@@ -46,6 +46,7 @@ def _state(hf, ctx):
     return [G, fields, count, acc] + [np.concatenate([np.ravel(x) for x in ob]) for ob in obs]
 
 
+@pytest.mark.parametrize("U", [0.0, 8.0, 16.0])      # 16: updates in FP64 arithmetic
 @pytest.mark.parametrize("L", LS)
 def test_a_run_in_several_launches_is_the_run_in_one(hf, L, U):
     """Split off the refreshes (after sweeps 10, 20 of a chain) and within a bin: bit for bit."""
