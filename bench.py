@@ -397,11 +397,12 @@ def run_reference(args):
 
 FP32_PEAK_TFLOPS = 2.0 * 128 * 152 * 2.07e9 / 1e12   # 128 FFMA/clk/SM
 DF_OPS_PER_FMA = 12          # FP32-pipe ops of one double-float multiply-add (lazy renormalisation)
-# DRAM bytes (read + write) of one full-size launch, from one ncu capture of the kernel built from
+# DRAM bytes (read + write) of one launch of all chains, from one ncu capture of the kernel built from
 # sources whose sha256 starts with the given prefix (the capture's command and counters are kept
-# in the profile summaries); a kernel whose sources changed since reports null.
-MEASURED_TRAFFIC = {"qmc_f64_kernel": (2295808 + 3584, "04c6f020ee92be69"),
-                    "qmc_df64_kernel": (2386432 + 3584, "5e3b37f3293b93e3"),
+# in the profile summaries; the two sweep kernels' launches of 40 sweeps move the chain state as their
+# full-length ones do); a kernel whose sources changed since reports null.
+MEASURED_TRAFFIC = {"qmc_f64_kernel": (5256192 + 225792, "709d78d8761707b9"),
+                    "qmc_df64_kernel": (2276352 + 6912, "5b39f08495a051d5"),
                     # the blocked lattice step, one launch of all 500 matrices: slab16 (N = 1024,
                     # b = 128) and box16p (N = 4096, b = 512)
                     "lattice_wide_kernel:slab16": (2160.4e6 + 2092.8e6, "9b62c014a9ceece6"),
@@ -446,6 +447,9 @@ def sweep_peak_tflops(form):
     """FP64-equivalent rate of the sweep arithmetic's own pipe."""
     return FX_PEAK_TFLOPS if form == 0 else FP32_PEAK_TFLOPS / DF_OPS_PER_FMA
 
+
+SWEEP_ARITHMETIC = {0: "64-bit fixed point, a unit per row, FP64 refreshes and near decisions",
+                    2: "FP32 pairs (48-bit significand), FP64 refreshes and near decisions"}
 
 FX_ROOF = ("serial two-pipe roof: refresh on FP64 (2 DFMA/clk/SM), then the 64-bit fixed-point sweeps "
            "on the integer pipe (2048 updates per 213 cycles and SM, probe), both at 2.07 GHz")
@@ -667,7 +671,10 @@ def run_ours(args):
             "data": "synthetic",
             "config": {"workload": WORKLOAD, "chains": nc * world, "time_slices": L,
                        "parallelism": "replicas%d" % world, "sweep_form": form,
-                       "team_warps": tw if tw else "default", "delay_k": dk,
+                       "sweep_arithmetic": SWEEP_ARITHMETIC.get(form),
+                       # (the fixed-point kernel's own: a warp per spin and four flips per pass)
+                       "team_warps": "1 per spin" if form == 0 else tw if tw else "default",
+                       "delay_k": 4 if form == 0 else dk,
                        "refresh_stagger": args.refresh_stagger,
                        "l2": "flushed (256 MB write) between timed steps"},
             "rdmft_iteration_ms": ms_per_step,
