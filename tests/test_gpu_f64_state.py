@@ -102,3 +102,57 @@ def test_a_measurement_is_the_sum_over_g(hf, L, U):
                 tol = 4 * 2.0 ** -53 * math.fsum(map(abs, x)) / L
                 assert abs(got[sp * L + m] - math.fsum(x) / L) <= tol, (i, sp, m)
     ctx.close()
+
+
+def test_a_batch_of_both_updates_is_its_problems_alone(hf):
+    """Rows of 57 and 59 bits, L = 64 and FP64 updates (dtau U > 3) in one captured iteration: every
+    problem's state and self-energy are those of its own iterations, bit for bit."""
+    import torch
+
+    stream = torch.cuda.Stream()
+    problems = [(16, 2.0), (32, 8.0), (64, 8.0), (20, 16.0), (64, 14.0)]
+    alone, fused = [], []
+    for group in (alone, fused):
+        for k, (L, U) in enumerate(problems):
+            cfg = dict(wl.CONFIGS["square6"], beta=0.25 * L, dtau=0.25, U=U, mu=U / 2, chains_per_site=3,
+                       n_warmup=4, n_measure=12, bin_size=4, max_bins=3, refresh_every=5, n_matsubara=64,
+                       seed=70 + k)
+            group.append(hf.Context(hf.make_params(cfg), stream=stream))
+    batch = hf.hf_batch_create([c.handle for c in fused], 1)
+    for _ in range(3):
+        hf.hf_batch_rdmft_step(batch)
+        for c in alone:
+            hf.hf_rdmft_step(c.handle)
+    for a, f in zip(alone, fused):
+        assert all(np.array_equal(x, y) for x, y in zip(_state(hf, a), _state(hf, f)))
+        assert np.array_equal(hf.hf_get_sigma(a.handle, a.n_sites, 64), hf.hf_get_sigma(f.handle, f.n_sites, 64))
+    hf.hf_batch_free(batch)
+    for c in alone + fused:
+        c.close()
+
+
+def test_served_solves_of_both_updates_share_a_launch(hf):
+    """The same request alone and among others of either form gives the same result."""
+    def server():
+        p = hf.hf_srv_params()
+        for k, v in dict(chains_per_request=4, n_warmup=6, n_measure=12, refresh_every=5, bin_size=4, precision=0,
+                         team_warps=0, max_L=64, max_inflight=32, max_keys=64, n_streams=2,
+                         requests_per_launch=16).items():
+            setattr(p, k, v)
+        return hf.Server(p)
+
+    def request(k, L, U):
+        return hf.make_request(0, k, L, 0.25 * L, U, 5, wl.random_baths(300 + k, 1, 0.25 * L, L)[0])
+
+    mix = [request(k, L, U) for k, (L, U) in enumerate([(16, 2.0), (20, 16.0), (64, 8.0), (64, 14.0), (32, 8.0)] * 3)]
+    s = server()
+    tickets = [hf.hf_srv_submit(s.handle, r) for r in mix]
+    together = [hf.hf_srv_wait(s.handle, t) for t in tickets]
+    s.close()
+    for r, want in zip(mix, together):
+        s = server()
+        got = hf.hf_srv_wait(s.handle, hf.hf_srv_submit(s.handle, r))
+        s.close()
+        for key in want:
+            if "latency" not in key and "ticket" not in key:
+                assert np.array_equal(np.asarray(want[key]), np.asarray(got[key])), key
